@@ -78,8 +78,8 @@ void release(qed_model *m) {
         if (p) cudaFree(p);
     split_release(m);
     adjoint_release(m);
-    sparse_release(m);
-    small_release(m);
+    sparse_release(m->sx);
+    small_release(m->small);
     for (auto &e : m->ev)
         if (e) cudaEventDestroy(e);
     delete m;
@@ -325,6 +325,7 @@ qed_status dense_propagator(qed_model *m, int scheme, cudaStream_t s) {
         QED_TRY(propagator(s, D, dt, m->work1, norm1, m->U, m->err));
     QED_CUDA_TRY(cudaMemcpy(&m->err_host, m->err, 4, cudaMemcpyDeviceToHost));
     if (m->err_host & kErrSingular) {
+        QED_CUDA_TRY(cudaMemset(m->err, 0, 4));
         set_error("singular Pade denominator");
         return QED_ENUMERIC;
     }
@@ -356,6 +357,44 @@ qed_status compute_propagator(qed_model *m, int scheme, cudaStream_t s) {
     }
     QED_CUDA_TRY(cudaMemcpy(m->phase, ph.data(), (size_t)D * 16, cudaMemcpyHostToDevice));
     return QED_OK;
+}
+
+// A new propagator of `scheme`, and what is derived from it, in place of m's: `make` forms U and its
+// tables in a model without any (U in the other buffer: the set-up writes work1, never work2).
+// If that fails the model is what it was, so that it steps on and the call can be repeated.  Nothing
+// of the model may be running.
+template <class Make>
+qed_status replace_propagator(qed_model *m, int32_t scheme, cudaStream_t s, Make make) {
+    SparseX *const sx = m->sx;
+    SmallModel *const small = m->small;
+    const bool strips = m->strips, u_ready = m->u_ready;
+    const int32_t old_scheme = m->scheme;
+    const std::vector<double2> phase = m->h_phase;
+    m->sx = nullptr;
+    m->small = nullptr;
+    m->strips = false;
+    m->scheme = scheme;
+    std::swap(m->U, m->work2);
+    qed_status st = make();
+    if (st == QED_OK && m->prec != QED_FP64) st = split_prepare(m, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (st == QED_OK) {
+        sparse_release(sx);
+        small_release(small);
+        QED_CUDA_TRY(e);
+        return QED_OK;
+    }
+    sparse_release(m->sx);
+    small_release(m->small);
+    m->sx = sx;
+    m->small = small;
+    m->strips = strips;
+    m->u_ready = u_ready;
+    m->scheme = old_scheme;
+    m->h_phase = phase;
+    std::swap(m->U, m->work2);
+    cudaMemcpy(m->phase, phase.data(), phase.size() * sizeof(double2), cudaMemcpyHostToDevice);
+    return st;
 }
 
 // Device side of a model whose host model m->host is built: operators, tables, U, and
@@ -625,13 +664,10 @@ qed_status qed_set_scheme(qed_model *m, int32_t scheme) {
     // the captured step graphs belong to the old scheme
     QED_CUDA_TRY(cudaDeviceSynchronize());
     drop_graphs(m);
-    const bool new_u = (scheme == QED_SCHEME_EFFECTIVE) != (m->scheme == QED_SCHEME_EFFECTIVE);
+    // the effective step has its own propagator, phases and (no) damping table
+    if ((scheme == QED_SCHEME_EFFECTIVE) != (m->scheme == QED_SCHEME_EFFECTIVE))
+        QED_TRY(replace_propagator(m, scheme, nullptr, [&] { return compute_propagator(m, scheme, nullptr); }));
     m->scheme = scheme;
-    if (new_u) {
-        // the effective step has its own propagator, phases and (no) damping table
-        QED_TRY(compute_propagator(m, scheme, nullptr));
-        if (m->prec != QED_FP64) QED_TRY(split_prepare(m, nullptr));
-    }
     split_set_scheme(m, scheme);
     QED_CUDA_TRY(cudaDeviceSynchronize());
     return QED_OK;
@@ -795,17 +831,15 @@ qed_status qed_sync_status(qed_model *m, qed_stream stream) {
 qed_status qed_set_U(qed_model *m, const void *U, qed_stream stream) {
     if (!m || !U) return einval("NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    QED_CUDA_TRY(cudaMemcpyAsync(m->U, U, (size_t)(m->D * m->D) * 16, cudaMemcpyDeviceToDevice, s));
-    // from here on the step is formed with this U, not with exp of the sparse H
     QED_CUDA_TRY(cudaDeviceSynchronize());
     drop_graphs(m);
-    sparse_release(m);
-    m->strips = false;
-    m->u_ready = true;
-    if (m->D <= kSmallMaxDim) QED_TRY(small_prepare(m, true, {}));
-    if (m->prec != QED_FP64) QED_TRY(split_prepare(m, s));
-    QED_CUDA_TRY(cudaStreamSynchronize(s));
-    return QED_OK;
+    // from here on the step is formed with this U, not with exp of the sparse H
+    return replace_propagator(m, m->scheme, s, [&]() -> qed_status {
+        QED_CUDA_TRY(cudaMemcpyAsync(m->U, U, (size_t)(m->D * m->D) * 16, cudaMemcpyDeviceToDevice, s));
+        QED_CUDA_TRY(cudaStreamSynchronize(s));
+        m->u_ready = true;
+        return m->D <= kSmallMaxDim ? small_prepare(m, true, {}) : QED_OK;
+    });
 }
 
 qed_status qed_get_U(const qed_model *m, void *U, qed_stream stream) {

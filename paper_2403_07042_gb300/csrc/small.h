@@ -30,10 +30,10 @@ struct SmallModel {
     const int32_t *in_ptr = nullptr, *in_jump = nullptr, *in_src = nullptr;
 };
 
-// Sets m->small where the model is small enough (and the device can hold the cluster), with the
+// Sets m->small (null before) where the model is small enough (and the device can hold the cluster), with the
 // components of H's graph, or every state for every row (`whole`: an injected U).
 qed_status small_prepare(qed_model *m, bool whole, const std::vector<int> &component);
-void small_release(qed_model *m);
+void small_release(SmallModel *a);
 // What a run records: the observables ids[0 .. n_obs) (as qed_evolve's) at every step whose
 // number, counted from `first`, is a multiple of `every`; rows of `out` from `row` on.
 struct SmallRecords {

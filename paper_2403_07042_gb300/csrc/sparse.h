@@ -64,12 +64,12 @@ constexpr double kSparseMaxNormF64 = 8.0;
 // step 22 us in passes, 9.2 us in products; the products pass 8 us each near dim 96).
 constexpr int kSparseMinDimF64 = 96;
 
-// Builds the tables of m's scheme from its host model (replacing older ones); m->sx stays
+// Builds the tables of m's scheme from its host model into m->sx, which is null before and stays
 // null where the series does not apply (the dense products then form the step).
 qed_status sparse_prepare(qed_model *m, int scheme);
 // The component of each state in H's graph (couplings of strength zero included).
 std::vector<int> hamiltonian_components(const HostModel &hm);
-void sparse_release(qed_model *m);
+void sparse_release(SparseX *x);
 
 void sparse_pass_f64(cudaStream_t s, const SparseX &x, const double2 *in, double2 *out, bool conj_side,
                      SparsePhase phases);

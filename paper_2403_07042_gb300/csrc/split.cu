@@ -964,9 +964,12 @@ void k_block_lists(const std::vector<uint8_t> &nz, int64_t D, int64_t Dp, const 
 // product runs unsplit, largest first, since the batch itself fills the GPU.  GEMM1 skips
 // tiles that lie wholly in the zero padding (rows or columns >= D); GEMM2 runs the tiles on
 // or above the diagonal only (its epilogue writes both halves of the Hermitian V).
-qed_status build_batch(Batch &b, qed_model *const *ms, int n, bool single, int batch_bn1 = kTcBNMax,
+// `target` is replaced at the end: a failed call leaves it as it was.
+qed_status build_batch(Batch &target, qed_model *const *ms, int n, bool single, int batch_bn1 = kTcBNMax,
                        int batch_bn2 = kTcBNMax) {
-    b.release();
+    struct Fresh : Batch {
+        ~Fresh() { release(); }
+    } b;
     b.n = n;
     b.scheme = ms[0]->scheme;
     for (int i = 1; i < n; ++i)
@@ -1150,6 +1153,9 @@ qed_status build_batch(Batch &b, qed_model *const *ms, int n, bool single, int b
         }
     }
     if (!tc_gemm_prepare_grouped()) return QED_ECUDA;
+    target.release();
+    target = b;
+    b.block = nullptr;
     return QED_OK;
 }
 
@@ -1280,6 +1286,36 @@ qed_status split_prepare(qed_model *m, cudaStream_t s) {
     }
     SplitState &S = *m->sp;
     const bool eff = m->scheme == QED_SCHEME_EFFECTIVE;
+    SPLIT_TRY(ensure_propagator(m, s));
+    // Delta into work1, its scales from a host copy, then the constant planes
+    make_delta_kernel<<<blocks_for(D * D, 256), 256, 0, s>>>(D, m->U, m->phase, m->work1, eff ? 0 : 1);
+    count_launches(1);
+    const int64_t nb = (D + 63) / 64;
+    QED_CUDA_TRY(cudaMemsetAsync(S.stats, 0, (size_t)(16 + nb * nb), s));
+    delta_stats_kernel<<<(unsigned)D, 256, 0, s>>>(D, m->work1, (unsigned long long *)S.stats, S.stats + 16);
+    count_launches(1);
+    std::vector<uint8_t> h((size_t)(16 + nb * nb));
+    QED_CUDA_TRY(cudaMemcpyAsync(h.data(), S.stats, h.size(), cudaMemcpyDeviceToHost, s));
+    QED_CUDA_TRY(cudaStreamSynchronize(s));
+    double maxabs = 0.0, maxrow = 0.0;
+    std::memcpy(&maxabs, h.data(), 8);
+    std::memcpy(&maxrow, h.data() + 8, 8);
+    // largest scaled magnitude 2^14 (FP16 max 65504); |rho_kl| <= 1, |W_kl| <= max row sum of |Delta|
+    const double scale_delta = S.scale_delta, scale_w = S.scale_w;
+    std::vector<uint8_t> nz(h.begin() + 16, h.end());
+    S.nz.swap(nz);
+    S.scale_delta = pow2_scale(maxabs, 14);
+    S.scale_rho = std::ldexp(1.0, 14);
+    S.scale_w = pow2_scale(maxrow, 14);
+    // the last that may run out of memory; the tables are written once it has not
+    qed_model *self[1] = {m};
+    const qed_status st = build_batch(S.self, self, 1, true);
+    if (st != QED_OK) {
+        S.nz.swap(nz);
+        S.scale_delta = scale_delta;
+        S.scale_w = scale_w;
+        return st;
+    }
     {
         // per-row phases P_k and dt/2 d_k (zero for the effective step, whose propagator holds
         // the anticommutator) as double-floats
@@ -1296,30 +1332,10 @@ qed_status split_prepare(qed_model *m, cudaStream_t s) {
         for (int64_t k = 0; k < D; ++k) damp[(size_t)k] = split_f(eff ? 0.0 : 0.5 * m->dt * anti[(size_t)k]);
         QED_CUDA_TRY(cudaMemcpy(S.damp_df, damp.data(), (size_t)D * sizeof(float2), cudaMemcpyHostToDevice));
     }
-    SPLIT_TRY(ensure_propagator(m, s));
-    // Delta into work1, its scales from a host copy, then the constant planes
-    make_delta_kernel<<<blocks_for(D * D, 256), 256, 0, s>>>(D, m->U, m->phase, m->work1, eff ? 0 : 1);
-    count_launches(1);
-    const int64_t nb = (D + 63) / 64;
-    QED_CUDA_TRY(cudaMemsetAsync(S.stats, 0, (size_t)(16 + nb * nb), s));
-    delta_stats_kernel<<<(unsigned)D, 256, 0, s>>>(D, m->work1, (unsigned long long *)S.stats, S.stats + 16);
-    count_launches(1);
-    std::vector<uint8_t> h((size_t)(16 + nb * nb));
-    QED_CUDA_TRY(cudaMemcpyAsync(h.data(), S.stats, h.size(), cudaMemcpyDeviceToHost, s));
-    QED_CUDA_TRY(cudaStreamSynchronize(s));
-    double maxabs = 0.0, maxrow = 0.0;
-    std::memcpy(&maxabs, h.data(), 8);
-    std::memcpy(&maxrow, h.data() + 8, 8);
-    S.nz.assign(h.begin() + 16, h.end());
-    // largest scaled magnitude 2^14 (FP16 max 65504); |rho_kl| <= 1, |W_kl| <= max row sum of |Delta|
-    S.scale_delta = pow2_scale(maxabs, 14);
-    S.scale_rho = std::ldexp(1.0, 14);
-    S.scale_w = pow2_scale(maxrow, 14);
     static_planes_kernel<<<blocks_for((int64_t)W2, 256), 256, 0, s>>>(D, Dp, m->work1, S.scale_delta, S.a1, S.b2);
     count_launches(1);
     QED_CUDA_TRY(cudaGetLastError());
-    qed_model *self[1] = {m};
-    return build_batch(S.self, self, 1, true);
+    return QED_OK;
 }
 
 qed_status split_begin(qed_model *m, const double2 *rho, bool check, cudaStream_t s) {
@@ -1480,11 +1496,17 @@ qed_status split_set_plan(qed_model *m, int bn1, int splits1, int bn2, int split
         set_error("qed_set_plan: more K slices than the product's 64-wide K blocks allow");
         return QED_EINVAL;
     }
-    S.g1 = g1;
-    S.g2 = g2;
+    std::swap(S.g1, g1);
+    std::swap(S.g2, g2);
+    const qed_status st = split_rebuild(m, s);
+    if (st != QED_OK) {
+        S.g1 = g1;
+        S.g2 = g2;
+        return st;
+    }
     S.batch_bn1 = bn1;
     S.batch_bn2 = bn2;
-    return split_rebuild(m, s);
+    return QED_OK;
 }
 
 void split_lindblad_stage(qed_model *m, int xsel, int bsel, int osel, float f, int planes, cudaStream_t s) {

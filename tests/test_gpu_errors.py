@@ -96,6 +96,59 @@ def test_alloc_budget_in_the_adjoint():
     assert abs(float(loss) - 1.0) <= 1e-6  # the trace of a closed unit-trace evolution
 
 
+def _same(model, rho0, rho_ref, u_ref):
+    rho = rho0.clone()
+    model.evolve(rho, 20)
+    model.sync()
+    return torch.equal(rho, rho_ref) and torch.equal(model.get_U(), u_ref)
+
+
+@pytest.mark.parametrize("precision,dim", [("fp64", 36), ("fp64", 70), ("fp64", 130), ("split_fp16x2", 130)])
+@pytest.mark.parametrize("change", ["effective", "lie", "U"])
+def test_failed_propagator_change_leaves_the_model_as_it_was(precision, dim, change):
+    """set_scheme and set_U that run out of memory at any of their allocations: the model steps on
+    with its old scheme and propagator, equal to the bit, and the repeated call takes effect."""
+    m = W.jch_two_cavities() if dim == 36 else W.chain_instance(np.random.default_rng(dim), dim, dim)
+    before, after = ("effective", "lie") if change == "lie" else ("lie", change)
+    gm, ref = (qed.Model(m, precision=precision, scheme=before) for _ in range(2))
+    rho0 = torch.from_numpy(W.random_density(dim, seed=3)).cuda()
+    other = torch.diag(torch.exp(1j * torch.arange(dim, device="cuda", dtype=torch.float64)))
+
+    def do(model):
+        if after == "U":
+            model.set_U(other)
+        else:
+            model.set_scheme(after)
+
+    def run(model):
+        rho = rho0.clone()
+        model.evolve(rho, 20)
+        model.sync()
+        return rho, model.get_U()
+
+    expected = run(ref)
+    do(ref)
+    changed = run(ref)
+    # (a change that allocates nothing new cannot fail)
+    failed, budget = 0, 0
+    while True:
+        qed.set_alloc_budget(budget)
+        try:
+            do(gm)
+            break
+        except qed.QedError as e:
+            assert e.status == qed.QED_ENOMEM
+            failed += 1
+        finally:
+            qed.set_alloc_budget(-1)
+        assert _same(gm, rho0, *expected), budget
+        budget = max(8 * dim, budget + budget // 2)
+        assert budget < 1 << 30
+    assert _same(gm, rho0, *changed)
+    if (precision, dim, after) != ("fp64", 130, "U") and (precision, dim, after) != ("fp64", 70, "U"):
+        assert failed > 0
+
+
 def test_alloc_budget_in_tc_gemm():
     A = torch.zeros((2, 128, 64), dtype=torch.float16, device="cuda")
     qed.set_alloc_budget(0)
