@@ -360,7 +360,7 @@ qed_status compute_propagator(qed_model *m, int scheme, cudaStream_t s) {
 }
 
 // A new propagator of `scheme`, and what is derived from it, in place of m's: `make` forms U and its
-// tables in a model without any (U in the other buffer: the set-up writes work1, never work2).
+// tables in a model without any (work2 keeps the old U: the set-up writes work1, never work2).
 // If that fails the model is what it was, so that it steps on and the call can be repeated.  Nothing
 // of the model may be running.
 template <class Make>
@@ -370,11 +370,12 @@ qed_status replace_propagator(qed_model *m, int32_t scheme, cudaStream_t s, Make
     const bool strips = m->strips, u_ready = m->u_ready;
     const int32_t old_scheme = m->scheme;
     const std::vector<double2> phase = m->h_phase;
+    const size_t bytes = (size_t)(m->D * m->D) * sizeof(double2);
+    if (u_ready) QED_CUDA_TRY(cudaMemcpyAsync(m->work2, m->U, bytes, cudaMemcpyDeviceToDevice, s));
     m->sx = nullptr;
     m->small = nullptr;
     m->strips = false;
     m->scheme = scheme;
-    std::swap(m->U, m->work2);
     qed_status st = make();
     if (st == QED_OK && m->prec != QED_FP64) st = split_prepare(m, s);
     const cudaError_t e = cudaStreamSynchronize(s);
@@ -392,7 +393,8 @@ qed_status replace_propagator(qed_model *m, int32_t scheme, cudaStream_t s, Make
     m->u_ready = u_ready;
     m->scheme = old_scheme;
     m->h_phase = phase;
-    std::swap(m->U, m->work2);
+    if (u_ready) cudaMemcpyAsync(m->U, m->work2, bytes, cudaMemcpyDeviceToDevice, s);
+    cudaStreamSynchronize(s);
     cudaMemcpy(m->phase, phase.data(), phase.size() * sizeof(double2), cudaMemcpyHostToDevice);
     return st;
 }
