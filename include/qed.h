@@ -24,7 +24,13 @@
  *
  * Density matrices are complex128, row-major, D x D, interleaved (re, im) — the layout
  * of a contiguous torch.complex128 tensor.  Rows and columns follow the basis order
- * returned by qed_basis_labels.
+ * returned by qed_basis_labels.  qed_evolve, qed_adjoint and qed_select_states of FP64 models,
+ * qed_set_U and qed_get_U take arrays aligned as a double is; split-precision models,
+ * qed_observables and qed_profile read 16-byte elements.
+ *
+ * A caller's CUDA graph that captured calls on a model holds that model's tables: it is
+ * captured again after qed_set_U, qed_set_scheme, qed_set_plan, qed_autotune and
+ * qed_set_wait_gate.
  */
 #ifndef QED_H
 #define QED_H

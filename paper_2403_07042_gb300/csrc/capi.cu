@@ -687,7 +687,17 @@ qed_status qed_evolve(qed_model *m, void *rho_v, int64_t n_steps, int64_t step_o
     double2 *rho = (double2 *)rho_v;
     const int64_t D = m->D;
     const bool split = m->prec != QED_FP64;
-    if (in_cluster(m)) return small_run(m, rho, n_steps, step_offset, record_every, n_obs, records, s);
+    if (in_cluster(m)) {
+        // its kernel moves rho as 16-byte elements; an array of doubles need not start on such a boundary
+        const bool aligned = (uintptr_t)rho % 16 == 0;
+        double2 *x = aligned ? rho : m->rho_int;
+        if (!aligned)
+            QED_CUDA_TRY(cudaMemcpyAsync(x, rho, (size_t)(D * D) * 16, cudaMemcpyDeviceToDevice, s));
+        QED_TRY(small_run(m, x, n_steps, step_offset, record_every, n_obs, records, s));
+        if (!aligned)
+            QED_CUDA_TRY(cudaMemcpyAsync(rho, x, (size_t)(D * D) * 16, cudaMemcpyDeviceToDevice, s));
+        return QED_OK;
+    }
     if (split) {
         QED_TRY(split_begin(m, rho, true, s));
     } else {
@@ -850,10 +860,14 @@ qed_status qed_get_U(const qed_model *m, void *U, qed_stream stream) {
     if (!m->u_ready) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         QED_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
-        if (capture != cudaStreamCaptureStatusNone && (uintptr_t)U % 16 == 0) {
-            // nothing runs now, so the model's own U stays to be formed
-            sparse_propagator(s, *m->sx, (double2 *)U, m->prec == QED_FP64);
+        if (capture != cudaStreamCaptureStatusNone) {
+            // nothing runs now, so the model's own U stays to be formed (the pass stores 16-byte elements)
+            const bool aligned = (uintptr_t)U % 16 == 0;
+            double2 *to = aligned ? (double2 *)U : m->work1;
+            sparse_propagator(s, *m->sx, to, m->prec == QED_FP64);
             QED_CUDA_TRY(cudaGetLastError());
+            if (!aligned)
+                QED_CUDA_TRY(cudaMemcpyAsync(U, to, (size_t)(m->D * m->D) * 16, cudaMemcpyDeviceToDevice, s));
             return QED_OK;
         }
         QED_TRY(ensure_propagator(const_cast<qed_model *>(m), s));

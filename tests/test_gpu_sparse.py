@@ -218,3 +218,42 @@ def test_fp64_propagator_is_exact_in_its_small_elements(D, detuned):
     size = np.hypot(re.astype(float), im.astype(float))[second]
     assert size.min() > 0
     assert (err / size).max() <= 32 * U
+
+
+@pytest.mark.parametrize("D", [2, 36, 64, 65, 130])
+def test_fp64_rho_need_not_start_on_a_16_byte_boundary(D):
+    """A complex array of a C program starts where a double may: every FP64 size takes it, and the
+    steps and records are those of an aligned copy, to the bit."""
+    import ctypes
+    gm = qed.Model(chain(D))
+    rho = state(D)
+    at = torch.zeros(2 * D * D + 3, dtype=torch.float64, device="cuda")
+    odd = at[1:1 + 2 * D * D]
+    assert odd.data_ptr() % 16 == 8
+    odd.copy_(torch.view_as_real(rho).reshape(-1))
+    ids = np.arange(D + 1, dtype=np.int32)
+    rec = torch.zeros((4, D + 1), dtype=torch.float64, device="cuda")
+    expected = gm.evolve(rho, 6, record_every=2, obs_ids=ids)
+    status = qed.lib().qed_evolve(gm._h, ctypes.c_void_p(odd.data_ptr()), 6, 0, 2, D + 1,
+                                  ids.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
+                                  ctypes.c_void_p(rec.data_ptr()),
+                                  ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert status == 0
+    gm.sync()
+    assert torch.equal(odd, torch.view_as_real(rho).reshape(-1)) and torch.equal(rec, expected)
+    assert at[0].item() == 0.0 and at[1 + 2 * D * D:].abs().max().item() == 0.0
+
+
+def test_captured_get_U_into_an_array_of_doubles():
+    """The same for a captured read of the late U."""
+    import ctypes
+    D = 130
+    gm, expected = qed.Model(chain(D)), qed.Model(chain(D)).get_U()
+    odd = torch.zeros(2 * D * D + 1, dtype=torch.float64, device="cuda")[1:]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        status = qed.lib().qed_get_U(gm._h, ctypes.c_void_p(odd.data_ptr()),
+                                     ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert status == 0
+    graph.replay()
+    assert torch.equal(odd, torch.view_as_real(expected).reshape(-1))
