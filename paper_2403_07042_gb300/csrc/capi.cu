@@ -382,6 +382,7 @@ qed_status replace_propagator(qed_model *m, int32_t scheme, cudaStream_t s, Make
     if (st == QED_OK) {
         sparse_release(sx);
         small_release(small);
+        adjoint_release(m);  // its backward model holds planes of the old U^+
         QED_CUDA_TRY(e);
         return QED_OK;
     }

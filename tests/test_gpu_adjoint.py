@@ -277,3 +277,32 @@ def test_split_adjoint_24x24_full_size_against_finite_differences():
         ref = (g["grad_g"] if name == "g" else g["grad_zeta"])[i]
         print(f"{name}[{i}]: adjoint {ad:.8e} fd {fd:.8e} oracle {ref:.8e}")
         assert abs(ad - fd) <= 1e-4 * abs(fd) + 1e-5, (name, i, ad, fd)
+
+
+@pytest.mark.parametrize("precision", ["split_fp16x2", "fp64"])
+def test_adjoint_follows_a_replaced_propagator(precision):
+    """Gradients of one model before and after set_U, and after its own propagator came back,
+    against models that only ever had the one U: equal bits (the backward model is made anew)."""
+    m = W.lattice(5, 4, seed=2, gamma=0.01, dt=0.1, start=(0, 0))
+    other = W.lattice(5, 4, seed=3, gamma=0.01, dt=0.1, start=(0, 0))
+    b = oracle.enumerate_basis(m)
+    rho0 = _cuda(oracle.initial_density(m, b))
+    w = _cuda(oracle.loss_diag(m, b, photons=[0, 1], atoms=[2]))
+    gm, own, given = (qed.Model(m, precision=precision) for _ in range(3))
+    U = qed.Model(other, precision=precision).get_U()
+    given.set_U(U)
+
+    def grads(model):
+        return [x.clone() for x in model.adjoint(rho0, 40, w, checkpoint_every=16)]
+
+    def same(x, y):
+        return all(torch.equal(p, q) for p, q in zip(x, y))
+
+    expected, injected = grads(own), grads(given)
+    assert same(grads(gm), expected)
+    assert not same(expected, injected)
+    gm.set_U(U)
+    assert same(grads(gm), injected)
+    gm.set_scheme("effective")
+    gm.set_scheme("lie")
+    assert same(grads(gm), expected)
