@@ -158,7 +158,8 @@ qed_status qed_spec_restricted(const qed_spec *spec, const int64_t *keep, int64_
  * split precision also prepares the
  * diagonal phase P = diag(exp(-i H_kk dt)), Delta = P^-1 U - I and its FP16 hi/lo
  * operand planes.  Synchronises `stream`.  EINVAL on a bad spec, ENOMEM, ECUDA,
- * ENUMERIC (non-finite U, singular Pade denominator), EUNSUPPORTED for reserved precisions. */
+ * ENUMERIC (a row of |H| or dt |H| that is not finite, singular Pade denominator),
+ * EUNSUPPORTED for reserved precisions. */
 qed_status qed_build(const qed_spec *spec, double dt, qed_precision prec, qed_stream stream,
                      qed_model **out);
 

@@ -337,6 +337,15 @@ qed_status compute_propagator(qed_model *m, int scheme, cudaStream_t s) {
     const int64_t D = m->D;
     const HostModel &hm = m->host;
     const bool eff = scheme == QED_SCHEME_EFFECTIVE;
+    // rows of |H|: one that is not finite, or not times dt, has no propagator (and no number of squarings)
+    std::vector<double> row((size_t)D, 0.0);
+    for (const auto &e : hm.h_entries) row[(size_t)e.row] += std::abs(entry_coefficient(hm, e) * e.unit);
+    for (int64_t k = 0; k < D; ++k)
+        if (!std::isfinite(row[(size_t)k]) ||
+            !std::isfinite(m->dt * row[(size_t)k] + (eff ? 0.5 * m->dt * hm.anti_diag[(size_t)k] : 0.0))) {
+            set_error("non-finite H or dt H");
+            return QED_ENUMERIC;
+        }
     m->u_ready = false;
     QED_TRY(sparse_prepare(m, scheme));
     m->strips = m->prec == QED_FP64 && m->sx && D >= kSparseMinDimF64;

@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const doubl
     double top = 0.0, sum = 0.0;
     for (int64_t l = threadIdx.x; l < D; l += blockDim.x) {
         const double2 d = Dl[k * D + l];
-        const double x = hypot(d.x, d.y);
+        double x = hypot(d.x, d.y);
+        if (!(x <= HUGE_VAL)) x = HUGE_VAL;  // NaN counts as infinity
         top = fmax(top, x);
         sum += x;
         if (d.x != 0.0 || d.y != 0.0) nz[(k / 64) * nb + l / 64] = 1;
@@ -183,9 +184,8 @@ __global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const doubl
         top = fmax(top, part[0][w]);
         sum += part[1][w];
     }
-    // (NaN counts as infinity)
-    atomicMax(&stats[0], (unsigned long long)__double_as_longlong(top == top ? top : HUGE_VAL));
-    atomicMax(&stats[1], (unsigned long long)__double_as_longlong(sum == sum ? sum : HUGE_VAL));
+    atomicMax(&stats[0], (unsigned long long)__double_as_longlong(top));
+    atomicMax(&stats[1], (unsigned long long)__double_as_longlong(sum));
 }
 
 // a1 = [[Dre, Dim], [Dim, -Dre]] and b2 = [[Dre, Dim], [-Dim, Dre]] (2Dp x 2Dp) as three

@@ -149,6 +149,20 @@ def test_failed_propagator_change_leaves_the_model_as_it_was(precision, dim, cha
         assert failed > 0
 
 
+@pytest.mark.parametrize("precision", ["fp64", "split_fp16x2"])
+@pytest.mark.parametrize("change", [dict(extra_tunnel=[float("nan")]), dict(extra_tunnel=[float("-inf")]),
+                                    dict(omega_c=1e308), dict(extra_tunnel=[1e300], dt=1e10),
+                                    dict(g=[1e308] * 4)])
+def test_hamiltonian_that_is_not_finite_is_refused(precision, change):
+    """A tunnelling amplitude that is not a number, or entries, row sums or dt H that overflow: no
+    propagator exists, in the series or in the Pade approximant."""
+    m = W.hb_shaped()
+    m.update(change)
+    with pytest.raises(qed.QedError) as ei:
+        qed.Model(m, precision=precision)
+    assert ei.value.status == qed.QED_ENUMERIC
+
+
 def test_alloc_budget_in_tc_gemm():
     A = torch.zeros((2, 128, 64), dtype=torch.float16, device="cuda")
     qed.set_alloc_budget(0)
