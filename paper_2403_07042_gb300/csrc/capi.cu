@@ -434,7 +434,7 @@ qed_status build_device(qed_model *m, double dt, qed_precision prec, cudaStream_
 
 qed_status ensure_propagator(qed_model *m, cudaStream_t s) {
     if (m->u_ready) return QED_OK;
-    sparse_propagator(s, *m->sx, m->U, m->prec == QED_FP64);
+    sparse_propagator(s, *m->sx, m->U);
     QED_CUDA_TRY(cudaGetLastError());
     // formed late, it may be read next from another stream
     if (m->strips) QED_CUDA_TRY(cudaStreamSynchronize(s));
@@ -874,7 +874,7 @@ qed_status qed_get_U(const qed_model *m, void *U, qed_stream stream) {
             // nothing runs now, so the model's own U stays to be formed (the pass stores 16-byte elements)
             const bool aligned = (uintptr_t)U % 16 == 0;
             double2 *to = aligned ? (double2 *)U : m->work1;
-            sparse_propagator(s, *m->sx, to, m->prec == QED_FP64);
+            sparse_propagator(s, *m->sx, to);
             QED_CUDA_TRY(cudaGetLastError());
             if (!aligned)
                 QED_CUDA_TRY(cudaMemcpyAsync(U, to, (size_t)(m->D * m->D) * 16, cudaMemcpyDeviceToDevice, s));

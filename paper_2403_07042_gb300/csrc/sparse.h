@@ -24,9 +24,8 @@ namespace qed {
 struct SparseX {
     void *block = nullptr;       // the allocation of every table
     int D = 0;
-    int width = 0;               // longest row
-    int terms = 0;               // Taylor terms of exp(X' / substeps)
-    int f64_terms = 0;           // the same for the FP64 loop, exact in small elements too
+    int terms = 0;               // Taylor terms of exp(X' / substeps) in a pass, exact in small elements too
+    int frechet_terms = 0;       // of the Frechet derivative's series
     int substeps = 0;
     double norm = 0.0;           // infinity norm of X'
     int *len = nullptr;          // [D] couplings of row k
@@ -34,13 +33,13 @@ struct SparseX {
     double *val = nullptr;       // [width][D]  dt H_kl
     double2 *diag = nullptr;     // [D] residual diagonal of X' (real, imaginary), or null if all zero
     double2 *phi = nullptr;      // [D] exp(Lambda_k)
-    // Rows sorted by their number of couplings (a warp's rows then end together), couplings as
-    // double-floats: entry j of sorted row p at [j * D + p].
-    int df_terms = 0;            // of `terms`, the first ones that need double-float sums
+    // Rows sorted by their number of couplings (a warp's rows then end together): entry j of sorted
+    // row p at [j * D + p].
     int2 *order = nullptr;       // [D] {row, couplings}
     int *place = nullptr;        // [D] the sorted place of row k
-    int4 *entry = nullptr;       // [max(width, 1)][D] {16 x column's place, dt H_kl's leading and trailing word, 0}
-    float4 *diag_df = nullptr;   // [D] {re hi, re lo, im hi, im lo}, or null
+    int4 *entry = nullptr;       // [longest row, at least 1][D] {column's place, 0, dt H_kl}
+    double *inv = nullptr;       // [terms + 1] 1 / (substeps n)
+    double2 *diag_sorted = nullptr;  // [D] diag in sorted order, or null
     // Lambda's distinct values: class of each row, and phi of class a times conj(phi) of b
     int *cls = nullptr;          // [D]
     double2 *pair = nullptr;     // [classes][classes], or null beyond kSparseClasses
@@ -87,7 +86,7 @@ void sparse_frechet(cudaStream_t s, const SparseX &x, const double2 *N, double2 
 // out = exp(X'), without the phases.
 void sparse_exp(cudaStream_t s, const SparseX &x, double2 *out);
 
-// m->U = exp(X) by one pass over the columns of the identity; `full`: in the FP64 loop.
-void sparse_propagator(cudaStream_t s, const SparseX &x, double2 *U, bool full);
+// U = exp(X) by one pass over the columns of the identity.
+void sparse_propagator(cudaStream_t s, const SparseX &x, double2 *U);
 
 }  // namespace qed

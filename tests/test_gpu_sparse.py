@@ -257,3 +257,53 @@ def test_captured_get_U_into_an_array_of_doubles():
     assert status == 0
     graph.replay()
     assert torch.equal(odd, torch.view_as_real(expected).reshape(-1))
+
+
+def _long_double_steps(m, n, k):
+    """(exp(-i H dt))^n e_k in long double, by the series of the whole H."""
+    H = np.asarray(qed.spec_hamiltonian(m)).real
+    X = H.astype(np.longdouble) * np.longdouble(m["dt"])
+    re, im = np.zeros(len(H), np.longdouble), np.zeros(len(H), np.longdouble)
+    re[k] = 1
+    for _ in range(n):
+        a, b = re.copy(), im.copy()
+        for j in range(1, 40):  # (-i X)^j / j! applied to a + i b
+            a, b = X @ b / j, -(X @ a) / j
+            re, im = re + a, im + b
+    return re, im
+
+
+@pytest.mark.parametrize("D,detuned", [(70, False), (96, True), (130, False), (257, True)])
+@pytest.mark.parametrize("n", [1, 4])
+def test_fp64_evolve_is_exact_in_its_small_elements(D, detuned, n):
+    """What couplings make out of a pure state, and out of a far smaller one in another component of
+    H, has the accuracy of its own size: U's elements up to second neighbours are within 32 u (the
+    test above), each side adds the roundings of a sum of up to 9 terms of one phase and of its
+    phases, so that a step takes 96 u of the element itself."""
+    m = chain(D, detuned)
+    m["jumps"] = []
+    H = np.asarray(qed.spec_hamiltonian(m)).real
+    near = ((H != 0) | (np.eye(D) > 0)).astype(int)
+    reach = near @ near > 0
+    joined = reach
+    for _ in range(10):
+        joined = joined @ joined
+    k = 1
+    far = np.flatnonzero(~joined[k])[-1]
+    small = 2.0 ** -100
+    rho = torch.zeros((D, D), dtype=torch.complex128, device="cuda")
+    rho[k, k], rho[far, far] = 1.0, small
+    gm = qed.Model(m)
+    gm.evolve(rho, n)
+    gm.sync()
+    got = rho.cpu().numpy()
+    for at, size in ((k, 1.0), (far, small)):
+        re, im = _long_double_steps(m, n, at)
+        of = np.flatnonzero(reach[at])
+        re, im = re[of], im[of]
+        ref_re, ref_im = np.outer(re, re) + np.outer(im, im), np.outer(im, re) - np.outer(re, im)
+        block = got[np.ix_(of, of)] / size
+        err = np.hypot((block.real - ref_re).astype(float), (block.imag - ref_im).astype(float))
+        ref = np.hypot(ref_re.astype(float), ref_im.astype(float))
+        assert ref.min() > 0
+        assert (err / ref).max() <= 96 * n * U, (at, (err / ref).max() / U)
