@@ -307,3 +307,46 @@ def test_fp64_evolve_is_exact_in_its_small_elements(D, detuned, n):
         ref = np.hypot(ref_re.astype(float), ref_im.astype(float))
         assert ref.min() > 0
         assert (err / ref).max() <= 96 * n * U, (at, (err / ref).max() / U)
+
+
+@pytest.mark.parametrize("dt", [1.0, 0.1, 1e-2, 1e-4, 1e-6])
+def test_hopping_gradients_keep_their_accuracy_at_small_steps(dt):
+    """The gradient of a hopping that the excitation reaches after two couplings is of the order
+    dt^4: the series of the derivative must reach it at every dt.  Against long double, relative to
+    the largest: the states and co-states of four steps carry 96 u a step each (test above), their
+    products and the two series' sums 64 u more: 900 u."""
+    D, n = 129, 4
+    m = chain(D)
+    m["jumps"], m["dt"] = [], dt
+    H = np.asarray(qed.spec_hamiltonian(m)).real
+    gm = qed.Model(m)
+    L, nc = gm.labels(), m["n_cavities"]
+    atom = [3 * c + 1 for c in range(nc)]
+    k = next(i for i in range(D) if L[i].sum() == 1 and L[i][atom[-1]] == 1)  # an atom of the last cavity
+    rho = torch.zeros((D, D), dtype=torch.complex128, device="cuda")
+    rho[k, k] = 1.0
+    o = torch.zeros(D, dtype=torch.float64, device="cuda")
+    o[k] = 1.0
+    got = gm.adjoint(rho, n, o, checkpoint_every=n)[2].cpu().numpy()
+    # in long double: psi_j forwards, chi_j backwards from e_k, and dL/dzeta =
+    # 2 Re [<chi_n | psi_n>^* sum_j <chi_n | U^(n-1-j) dU psi_j>], dU by its series
+    X = H.astype(np.longdouble) * np.longdouble(dt)
+    grad = []
+    for b in range(len(m["zeta"])):
+        one = dict(m, g=[0.0] * len(m["g"]), zeta=[float(i == b) for i in range(len(m["zeta"]))], omega_c=0.0,
+                   omega_a=0.0)
+        E = np.asarray(qed.spec_hamiltonian(one)).real.astype(np.longdouble) * np.longdouble(dt)
+        # the pair (psi, dpsi) under exp(-i [[X, 0], [E, X]])
+        p = [np.zeros(D, np.longdouble) for _ in range(4)]
+        p[0][k] = 1
+        for _ in range(n):
+            t = [x.copy() for x in p]
+            for j in range(1, 40):
+                re, im, dre, dim = t
+                t = [X @ im / j, -(X @ re) / j, (X @ dim + E @ im) / j, -(X @ dre + E @ re) / j]
+                p = [x + y for x, y in zip(p, t)]
+        grad.append(2 * (p[0][k] * p[2][k] + p[1][k] * p[3][k]))
+    ref = np.array(grad)
+    size = float(np.abs(ref).max())
+    assert size > 0
+    assert float(np.abs(got - ref).max()) <= 900 * U * size, float(np.abs(got - ref).max()) / size / U
