@@ -20,11 +20,8 @@ struct SmallModel {
     size_t smem = 0;
     void *block = nullptr;  // the allocation of the tables below
     int *ptr = nullptr, *idx = nullptr;  // states of row i's component: idx[ptr[i] .. ptr[i + 1])
-    // exp(X') - I as FP32 words {re, im, re lo, im lo} (sparse.h), or null: the sums then run in FP64
-    // with the whole U
-    float4 *delta = nullptr;
     // of the model, filled in at launch
-    const double2 *U = nullptr, *phi = nullptr;
+    const double2 *U = nullptr;
     double dt = 0.0;
     const double *anti = nullptr, *in_coef = nullptr;
     const int32_t *in_ptr = nullptr, *in_jump = nullptr, *in_src = nullptr;

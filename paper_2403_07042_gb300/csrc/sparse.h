@@ -83,9 +83,6 @@ void sparse_conjugate_f64(cudaStream_t s, const SparseX &x, const double2 *in, d
 // away).  Each term is one sparse product from the left and one from the right.  work: 5 D x D.
 void sparse_frechet(cudaStream_t s, const SparseX &x, const double2 *N, double2 *G, double2 *work);
 
-// out = exp(X'), without the phases.
-void sparse_exp(cudaStream_t s, const SparseX &x, double2 *out);
-
 // U = exp(X) by one pass over the columns of the identity.
 void sparse_propagator(cudaStream_t s, const SparseX &x, double2 *U);
 

@@ -273,7 +273,8 @@ def _long_double_steps(m, n, k):
     return re, im
 
 
-@pytest.mark.parametrize("D,detuned", [(70, False), (96, True), (130, False), (257, True)])
+@pytest.mark.parametrize("D,detuned", [(8, False), (33, False), (64, True), (70, False), (96, True), (130, False),
+                                       (257, True)])
 @pytest.mark.parametrize("n", [1, 4])
 def test_fp64_evolve_is_exact_in_its_small_elements(D, detuned, n):
     """What couplings make out of a pure state, and out of a far smaller one in another component of
