@@ -27,7 +27,7 @@ struct SmallModel {
     const int32_t *in_ptr = nullptr, *in_jump = nullptr, *in_src = nullptr;
 };
 
-// Sets m->small (null before) where the model is small enough (and the device can hold the cluster), with the
+// Sets m->small (null before) where a cluster run pays (and the device can hold the cluster), with the
 // components of H's graph, or every state for every row (`whole`: an injected U).
 qed_status small_prepare(qed_model *m, bool whole, const std::vector<int> &component);
 void small_release(SmallModel *a);

@@ -103,12 +103,14 @@ def _same(model, rho0, rho_ref, u_ref):
     return torch.equal(rho, rho_ref) and torch.equal(model.get_U(), u_ref)
 
 
-@pytest.mark.parametrize("precision,dim", [("fp64", 36), ("fp64", 70), ("fp64", 130), ("split_fp16x2", 130)])
+@pytest.mark.parametrize("precision,dim", [("fp64", 8), ("fp64", 36), ("fp64", 70), ("fp64", 130),
+                                           ("split_fp16x2", 130)])
 @pytest.mark.parametrize("change", ["effective", "lie", "U"])
 def test_failed_propagator_change_leaves_the_model_as_it_was(precision, dim, change):
     """set_scheme and set_U that run out of memory at any of their allocations: the model steps on
     with its old scheme and propagator, equal to the bit, and the repeated call takes effect."""
-    m = W.jch_two_cavities() if dim == 36 else W.chain_instance(np.random.default_rng(dim), dim, dim)
+    m = {8: lambda: W.jc_single(n_max=3, g=0.02, dt=0.1, gamma=1e-3), 36: W.jch_two_cavities}.get(
+        dim, lambda: W.chain_instance(np.random.default_rng(dim), dim, dim))()
     before, after = ("effective", "lie") if change == "lie" else ("lie", change)
     gm, ref = (qed.Model(m, precision=precision, scheme=before) for _ in range(2))
     rho0 = torch.from_numpy(W.random_density(dim, seed=3)).cuda()
@@ -129,7 +131,6 @@ def test_failed_propagator_change_leaves_the_model_as_it_was(precision, dim, cha
     expected = run(ref)
     do(ref)
     changed = run(ref)
-    # (a change that allocates nothing new cannot fail)
     failed, budget = 0, 0
     while True:
         qed.set_alloc_budget(budget)
@@ -145,8 +146,8 @@ def test_failed_propagator_change_leaves_the_model_as_it_was(precision, dim, cha
         budget = max(8 * dim, budget + budget // 2)
         assert budget < 1 << 30
     assert _same(gm, rho0, *changed)
-    if (precision, dim, after) != ("fp64", 130, "U") and (precision, dim, after) != ("fp64", 70, "U"):
-        assert failed > 0
+    # (a given U needs tables of its own in a cluster run and in split precision)
+    assert failed > 0 or (precision == "fp64" and after == "U" and dim > 8)
 
 
 @pytest.mark.parametrize("precision", ["fp64", "split_fp16x2"])

@@ -351,3 +351,19 @@ def test_hopping_gradients_keep_their_accuracy_at_small_steps(dt):
     size = float(np.abs(ref).max())
     assert size > 0
     assert float(np.abs(got - ref).max()) <= 900 * U * size, float(np.abs(got - ref).max()) / size / U
+
+
+@pytest.mark.parametrize("D,injected,in_cluster", [(8, False, True), (8, True, True), (36, False, True),
+                                                   (36, True, False), (49, False, False), (64, True, False)])
+def test_fp64_runs_in_a_cluster_where_that_is_faster(D, injected, in_cluster):
+    """One launch a run, or three a step (long components of H, an injected U); the same results."""
+    gm = qed.Model(chain(D))
+    if injected:
+        gm.set_U(gm.get_U())
+    rho = state(D)
+    ref = rho.clone()
+    before = qed.launch_count()
+    gm.evolve(rho, 6)
+    assert qed.launch_count() - before == (1 if in_cluster else 18)
+    gm.profile(ref, 6)  # kernel by kernel
+    assert (rho - ref).abs().max().item() <= 6 * (4 * D + 64) * U
