@@ -52,8 +52,9 @@ void take_block(cudaStream_t s, int64_t D, int64_t W, int64_t c0, const double2 
 void take_right_half(cudaStream_t s, int64_t D, const double2 *aug, double2 *R);
 
 // Jump entries by row: entries [ptr[k], ptr[k + 1]) of row k, sorted by jump (incoming ones for the
-// forward map: source and coefficient), and the rows' jumps as bits (null: more than 32 jumps, or
-// one twice in a row).
+// forward map: source and coefficient), and the rows' jumps as bits (null: more than 32 jumps, more
+// than kJumpMaskEntries of them in a row, or one twice in a row).
+constexpr int kJumpMaskEntries = 16;
 struct JumpLists {
     const int32_t *ptr, *jump, *src;
     const double *coef;

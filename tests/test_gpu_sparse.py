@@ -367,3 +367,22 @@ def test_fp64_runs_in_a_cluster_where_that_is_faster(D, injected, in_cluster):
     assert qed.launch_count() - before == (1 if in_cluster else 18)
     gm.profile(ref, 6)  # kernel by kernel
     assert (rho - ref).abs().max().item() <= 6 * (4 * D + 64) * U
+
+
+@pytest.mark.parametrize("shape", [(3, 5), (4, 4), (17, 1), (5, 5), (8, 4), (11, 3)])
+@pytest.mark.parametrize("scheme", ["lie", "strang"])
+def test_fp64_jumps_into_one_state(shape, scheme):
+    """15 to 33 leaks into the vacuum, about the number that masks of the jumps take, against the
+    oracle with its own U."""
+    import oracle
+    m = W.lattice(*shape, gamma=0.02, seed=1)
+    b = oracle.enumerate_basis(m)
+    gm = qed.Model(m, scheme=scheme)
+    propagator = oracle.propagator(oracle.hamiltonian(m, b), m["dt"])
+    gm.set_U(torch.from_numpy(propagator).cuda())
+    rho0 = W.random_density(b.dim, seed=2)
+    rho = torch.from_numpy(rho0).cuda()
+    gm.evolve(rho, 30)
+    gm.sync()
+    ref = oracle.evolve(m, rho0=rho0, n_steps=30, U=propagator, basis=b, return_records=False, scheme=scheme)
+    assert np.abs(rho.cpu().numpy() - ref).max() <= 1e-12
