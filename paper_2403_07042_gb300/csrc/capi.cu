@@ -350,7 +350,7 @@ qed_status compute_propagator(qed_model *m, int scheme, cudaStream_t s) {
         }
     m->u_ready = false;
     QED_TRY(sparse_prepare(m, scheme));
-    m->strips = m->prec == QED_FP64 && m->sx && D >= kSparseMinDimF64;
+    m->strips = m->prec == QED_FP64 && D > kSmallMaxDim && m->sx && m->sx->pays;
     if (!m->sx)
         QED_TRY(dense_propagator(m, scheme, s));
     else if (!m->strips)

@@ -28,6 +28,7 @@ struct SparseX {
     int frechet_terms = 0;       // of the Frechet derivative's series
     int substeps = 0;
     double norm = 0.0;           // infinity norm of X'
+    bool pays = false;           // a step is faster through it (passes_pay)
     int *len = nullptr;          // [D] couplings of row k
     int *col = nullptr;          // [width][D]
     double *val = nullptr;       // [width][D]  dt H_kl
@@ -54,14 +55,24 @@ constexpr int kSparseClasses = 32;
 // kPhaseConj is kPhaseBoth conjugated, for U^+ In U.
 enum SparsePhase { kPhaseNone = 0, kPhaseBoth = 1, kPhaseRow = 2, kPhaseConj = 3 };
 
-// Largest dimension the FP64 kernel takes (one column's three buffers in shared memory) and the
-// largest norm of X' the series is used for.
+// Largest dimension a pass takes (three columns in shared memory), and the largest norm of X' that
+// the series is used for: eight substeps of 18 terms, where U costs half of a step's passes (below)
+// against ten and more dense products and an elimination.
 constexpr int kSparseMaxDimF64 = 4800;
 constexpr double kSparseMaxNormF64 = 8.0;
-// Below this dimension an FP64 step is two dense products: a pass takes 8 us however small the
-// model (6 dependent terms of an FP64 latency each), a small dense product less (dim 36: a
-// step 22 us in passes, 9.2 us in products; the products pass 8 us each near dim 96).
-constexpr int kSparseMinDimF64 = 96;
+
+// Whether V = U rho U^+ is faster in two passes than in two dense FP64 products, by estimates of a
+// step in us (Lindblad update and launches in both), fitted to chains of 65 to 801 states, lattices
+// of 73 to 1153 and single cavities with 64 atoms each at norms of 0.001 to 7.9 (6 to 144 terms):
+// within 20 %, and on the slower side only where both are equal (96 states).  A pass and term costs
+// its longest row's chain and the FP64 instructions of its couplings.  Passes and products, measured:
+// dim 96 and norm 0.05 27 and 20 us, dim 129 28 and 41; at norm 1.5 dim 160 96 and 67, dim 257 141
+// and 244; at norm 7.9 dim 350 935 and 642, dim 512 1860 and 2170; two cavities of 64 atoms (rows
+// of 65 couplings, dim 131, norm 0.05) 123 and 42, nine (dim 586) 183 and 4060.
+inline bool passes_pay(double D, double couplings, double longest, double terms) {
+    const double passes = 8.6 + 3.2e-5 * D * D + terms * (0.32 + 0.177 * longest + 6.9e-6 * D * (couplings + D));
+    return passes < 8.0 + 1.58e-5 * D * D * D;
+}
 
 // Builds the tables of m's scheme from its host model into m->sx, which is null before and stays
 // null where the series does not apply (the dense products then form the step).

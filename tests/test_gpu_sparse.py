@@ -386,3 +386,85 @@ def test_fp64_jumps_into_one_state(shape, scheme):
     gm.sync()
     ref = oracle.evolve(m, rho0=rho0, n_steps=30, U=propagator, basis=b, return_records=False, scheme=scheme)
     assert np.abs(rho.cpu().numpy() - ref).max() <= 1e-12
+
+
+def strong(D, norm):
+    """A chain whose couplings take the infinity norm of dt H without its diagonal to `norm`."""
+    m = chain(D)
+    for _ in range(2):
+        H = np.asarray(qed.spec_hamiltonian(m)).real * m["dt"]
+        now = np.abs(H - np.diag(np.diag(H))).sum(1).max()
+        m["g"], m["zeta"] = [x * norm / now for x in m["g"]], [x * norm / now for x in m["zeta"]]
+    assert abs(now - norm) <= 1e-12 * norm
+    return m
+
+
+@pytest.mark.parametrize("D,norm,scheme,passes", [
+    (33, 1.5, "lie", False), (33, 7.9, "effective", False), (64, 4.0, "lie", False), (130, 0.9, "lie", False),
+    (130, 1.5, "strang", False), (160, 0.9, "lie", True), (257, 1.5, "effective", True), (257, 4.0, "lie", False),
+    (350, 4.0, "strang", True), (512, 7.9, "lie", True), (33, 9.5, "lie", False), (130, 9.5, "effective", False),
+    (130, 40.0, "lie", False)])
+def test_fp64_strong_couplings_match_oracle(D, norm, scheme, passes):
+    """Norms of one to eight substeps and beyond the series (the Pade approximant, with squarings at
+    40), through passes or dense products as passes_pay has it, against the oracle with its own
+    propagator (an eigendecomposition; scipy's expm for the effective step).  U: a substep's sums are
+    within 30 u of the column (e times 11 roundings a term), eight of them 240 u, squarings double
+    what Pade and its elimination leave (D u); either reference is within 16 D u.  A step adds 4 D + 64."""
+    import oracle
+    m = strong(D, norm)
+    b = oracle.enumerate_basis(m)
+    H, jumps = oracle.hamiltonian(m, b), oracle.jump_operators(m, b)
+    ref_U = oracle.effective_propagator(H, jumps, m["dt"]) if scheme == "effective" else oracle.propagator(H, m["dt"])
+    gm = qed.Model(m, scheme=scheme)
+    bound = (256 + 16 * D * max(1.0, norm / 8)) * U
+    assert np.abs(gm.get_U().cpu().numpy() - ref_U).max() <= bound
+    n = 3
+    rho0 = W.random_density(D, seed=D)
+    ref = oracle.evolve(m, rho0=rho0, n_steps=n, U=ref_U, basis=b, return_records=False, scheme=scheme)
+    rho = torch.from_numpy(rho0).cuda()
+    gm.evolve(rho, n)
+    gm.sync()
+    assert np.abs(rho.cpu().numpy() - ref).max() <= n * (2 * bound + (4 * D + 64) * U)
+    assert ("strip_f64_1" in gm.profile(rho, 1)) == passes
+
+
+@pytest.mark.parametrize("D,norm,scheme", [(33, 1.5, "lie"), (33, 9.5, "strang"), (130, 1.5, "lie"), (130, 4.0, "strang"),
+                                           (257, 1.5, "lie")])
+def test_gradients_of_strong_couplings_match_oracle(D, norm, scheme):
+    """Beyond the first substep the derivative is the dense one, the co-state by passes (dim 257) or
+    products; to the FP64 adjoint's accuracy."""
+    import oracle
+    m = strong(D, norm)
+    b = oracle.enumerate_basis(m)
+    o = np.linspace(-1.0, 1.0, D)
+    rho0 = W.random_density(D, seed=D + 1)
+    ref = oracle.adjoint_gradients(m, o, n_steps=4, rho0=rho0, basis=b, scheme=scheme)
+    gm = qed.Model(m, scheme=scheme)
+    got = gm.adjoint(torch.from_numpy(rho0).cuda(), 4, torch.from_numpy(o).cuda(), checkpoint_every=3)
+    for x, y in zip(got[1:], ref[1:]):
+        y = np.asarray(y, float)
+        assert np.abs(x.cpu().numpy() - y).max() <= 1e-9 * np.abs(y).max()
+
+
+@pytest.mark.parametrize("shape", [(43, 43), (44, 54)])
+def test_fp64_passes_of_the_largest_dimensions(shape):
+    """3699 and 4753 states (the largest take 4800): a pure state's step, to the bound of 96 u of the
+    unit vector's projector."""
+    m = W.lattice(*shape, seed=5, gamma=0.0)
+    gm = qed.Model(m)
+    D = gm.dim
+    H = np.asarray(qed.spec_hamiltonian(m)).real * m["dt"]
+    k = D // 2
+    re, im = np.zeros(D), np.zeros(D)
+    re[k] = 1.0
+    a, b = re.copy(), im.copy()
+    for j in range(1, 25):
+        a, b = H @ b / j, -(H @ a) / j
+        re, im = re + a, im + b
+    psi = torch.from_numpy(re + 1j * im).cuda()
+    rho = torch.zeros((D, D), dtype=torch.complex128, device="cuda")
+    rho[k, k] = 1.0
+    gm.evolve(rho, 1)
+    gm.sync()
+    assert (rho - torch.outer(psi, psi.conj())).abs().max().item() <= 96 * U
+    assert "strip_f64_1" in gm.profile(rho, 1)
