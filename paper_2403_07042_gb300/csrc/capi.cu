@@ -825,7 +825,14 @@ qed_status qed_evolve_batched(int32_t n, qed_model *const *ms, void *const *rhos
     split_batch_destroy(b);
     if (st != QED_OK) return st;
     if (end != QED_OK) return end;
-    for (uint32_t e : errors) QED_TRY(status_of(e));
+    // the first failing instance's error is reported here, those behind it stay for their own
+    // qed_sync_status
+    for (int32_t i = 0; i < n; ++i) {
+        ms[i]->err_host = errors[(size_t)i];
+        if (errors[(size_t)i] == 0) continue;
+        QED_CUDA_TRY(cudaMemset(ms[i]->err, 0, 4));
+        return status_of(errors[(size_t)i]);
+    }
     return QED_OK;
 }
 

@@ -335,10 +335,10 @@ __global__ void __launch_bounds__(256) end_kernel(const TileItem *__restrict__ t
     }
 }
 
-// out[i] = instance i's error word, which becomes zero.
-__global__ void take_errors_kernel(int n, const InstDesc *__restrict__ descs, uint32_t *out) {
+// out[i] = instance i's error word.
+__global__ void read_errors_kernel(int n, const InstDesc *__restrict__ descs, uint32_t *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = atomicExch(descs[i].err, 0u);
+    if (i < n) out[i] = *descs[i].err;
 }
 
 // One block per instance: its populations into row `row` of its records.
@@ -1666,7 +1666,7 @@ void split_batch_populations(const Batch *b, int64_t row, cudaStream_t s) {
 
 qed_status split_batch_end(const Batch *b, std::vector<uint32_t> &errors, cudaStream_t s) {
     end_kernel<<<b->n_pairs, dim3(32, 8), 0, s>>>(b->pairs, b->desc, (double2 *const *)b->rhos, nullptr);
-    take_errors_kernel<<<blocks_for(b->n, 256), 256, 0, s>>>(b->n, b->desc, b->errors);
+    read_errors_kernel<<<blocks_for(b->n, 256), 256, 0, s>>>(b->n, b->desc, b->errors);
     count_launches(2);
     errors.assign((size_t)b->n, 0u);
     QED_CUDA_TRY(cudaMemcpyAsync(errors.data(), b->errors, (size_t)b->n * 4, cudaMemcpyDeviceToHost, s));

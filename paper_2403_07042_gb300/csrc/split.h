@@ -47,7 +47,7 @@ struct Batch;
 qed_status split_batch_create(qed_model *const *ms, int n, Batch **out);
 // The batch's split_begin (rhos, records: host arrays of device pointers; records may be null), a
 // row of every instance's populations, and the end: the states back into the rhos and every
-// instance's error word, which becomes zero.  split_batch_end synchronises `s`.
+// instance's error word read.  split_batch_end synchronises `s`.
 qed_status split_batch_begin(const Batch *b, void *const *rhos, double *const *records, cudaStream_t s);
 void split_batch_populations(const Batch *b, int64_t row, cudaStream_t s);
 qed_status split_batch_end(const Batch *b, std::vector<uint32_t> &errors, cudaStream_t s);

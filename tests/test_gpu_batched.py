@@ -212,3 +212,26 @@ def test_batched_argument_errors():
     with pytest.raises(qed.QedError) as ei:
         qed.evolve_batched(models, [rhos[0], bad], 5)
     assert ei.value.status == qed.QED_EINVAL
+
+
+def test_batched_errors_stay_with_their_instances():
+    """Two rejected matrices in a batch: the call reports the first one's, the second one's waits for
+    that model's own sync, and the good instance is evolved."""
+    ms = [W.chain_instance(np.random.default_rng(q), 33 + q, 33 + q) for q in range(3)]
+    models = [qed.Model(m, precision="split_fp16x2") for m in ms]
+    rhos = [torch.from_numpy(W.random_density(g.dim, seed=q)).cuda() for q, g in enumerate(models)]
+    single = rhos[0].clone()
+    for rho in rhos[1:]:
+        rho[0, 1] += 1e-3
+    with pytest.raises(qed.QedError) as ei:
+        qed.evolve_batched(models, rhos, 4)
+    assert ei.value.status == qed.QED_EINVAL
+    models[0].sync()
+    models[1].sync()  # reported above
+    with pytest.raises(qed.QedError) as ei:
+        models[2].sync()
+    assert ei.value.status == qed.QED_EINVAL
+    models[2].sync()
+    models[0].evolve(single, 4)
+    models[0].sync()
+    assert (single - rhos[0]).abs().max().item() <= 1e-7
