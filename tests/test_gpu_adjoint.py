@@ -306,3 +306,27 @@ def test_adjoint_follows_a_replaced_propagator(precision):
     gm.set_scheme("effective")
     gm.set_scheme("lie")
     assert same(grads(gm), expected)
+
+
+def test_kept_work_space_is_bounded_over_all_models():
+    """Gradients of three models whose work spaces (more than 1 GB each: 40 states of 1153 x 1153) stay
+    below the bound one by one, not together: what they keep is below it, and comes back with them."""
+    import gc
+    m = W.lattice(24, 24, seed=0)
+    b = oracle.enumerate_basis(m)
+    rho0, w = _cuda(oracle.initial_density(m, b)), torch.ones(b.dim, dtype=torch.float64, device="cuda")
+    models = [qed.Model(m) for _ in range(3)]
+    gc.collect()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    for gm in models:
+        gm.adjoint(rho0, 20, w, checkpoint_every=20)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert 1 << 30 < kept <= (2 << 30) + (64 << 20)
+    for gm in models:
+        gm.close()
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] >= free
