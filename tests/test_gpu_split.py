@@ -391,3 +391,35 @@ def test_profile_replay():
     with pytest.raises(qed.QedError) as ei:
         g64.profile_replay(before, 5)
     assert ei.value.status == qed.QED_EUNSUPPORTED
+
+
+def _many_jumps(D):
+    """Photon loss of five cavities, decay of their ten atoms: 15 jumps, 15 of them into the vacuum."""
+    m = W.chain_instance(np.random.default_rng(D), 64, 64)
+    rng = np.random.default_rng(D + 1)
+    m.update(n_cavities=5, atoms_per_cavity=[2] * 5, n_max=[2] * 5, dim_cap=D, dt=0.1,
+             g=[float(x) for x in rng.uniform(0.005, 0.02, size=10)], bonds=[(c, c + 1) for c in range(4)],
+             zeta=[float(x) for x in rng.uniform(0.002, 0.01, size=4)],
+             jumps=[(0, c, float(rng.uniform(0.01, 0.03))) for c in range(5)]
+             + [(1, a, float(rng.uniform(0.01, 0.03))) for a in range(10)])
+    return m
+
+
+@pytest.mark.parametrize("make", [
+    lambda: W.lattice(3, 3, gamma=0.02, seed=1), lambda: W.lattice(4, 4, gamma=0.02, seed=1),
+    lambda: W.lattice(17, 1, gamma=0.02, seed=1), lambda: W.lattice(8, 4, gamma=0.02, seed=1),
+    lambda: W.lattice(11, 3, gamma=0.02, seed=1), lambda: _many_jumps(63), lambda: _many_jumps(130)])
+@pytest.mark.parametrize("scheme", ["lie", "strang"])
+def test_updates_by_jump_masks(make, scheme):
+    """Rows with more entries than a block stages (9 to 16 jumps into one state), lists at the masks'
+    limits and past them (17 entries, 32 and 33 jumps): one lost or doubled jump moves an element by
+    30 dt gamma / D, 1e-4 and more; the step's own contract is 1e-5."""
+    m = make()
+    b = oracle.enumerate_basis(m)
+    gm = qed.Model(m, precision="split_fp16x2", scheme=scheme)
+    rho0 = W.random_density(b.dim, seed=4)
+    rho = torch.from_numpy(rho0).cuda()
+    gm.evolve(rho, 30)
+    gm.sync()
+    ref = oracle.evolve(m, rho0=rho0, n_steps=30, basis=b, return_records=False, scheme=scheme)
+    assert np.abs(rho.cpu().numpy() - ref).max() <= 1e-5
