@@ -367,8 +367,10 @@ qed_status qed_set_wait_gate(qed_model *m, int32_t closed, int64_t budget_cycles
 qed_status qed_set_alloc_budget(int64_t bytes);
 
 /*
- * Run n_steps steps like qed_evolve (no records), timing each kernel class with CUDA
- * events on `stream`; writes the mean duration in milliseconds per step of each class
+ * Run n_steps steps of qed_evolve (no records) kernel by kernel, timing each kernel class
+ * with CUDA events on `stream`.  An FP64 model of up to 64 states whose runs qed_evolve makes
+ * in one launch is stepped here by the three kernels of larger models (the same step, not
+ * qed_evolve's time).  Writes the mean duration in milliseconds per step of each class
  * into ms[0..n_kernels-1] and the class names (comma separated) into names (size
  * name_cap).  Synchronises.  For measurement only: it perturbs the pipelining.
  */
