@@ -292,23 +292,24 @@ __device__ bool long_merge_f64(int64_t D, const double2 *X, const int32_t *in_ju
                 sx = fma(c, g.x, sx);
                 sy = fma(c, g.y, sy);
             }
-        } else
-        for (int e = s0 + lane; e < s1; e += 32) {
-            const int j = in_jump[e];
-            int lo = l0, hi = l1;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (in_jump[mid] < j)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            if (lo < l1 && in_jump[lo] == j) {
-                const int ep = m_short ? e : lo, eq = m_short ? lo : e;
-                const double c = scale * in_coef[ep] * in_coef[eq];
-                const double2 g = X[(int64_t)in_src[ep] * D + in_src[eq]];
-                sx = fma(c, g.x, sx);
-                sy = fma(c, g.y, sy);
+        } else {
+            for (int e = s0 + lane; e < s1; e += 32) {
+                const int j = in_jump[e];
+                int lo = l0, hi = l1;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (in_jump[mid] < j)
+                        lo = mid + 1;
+                    else
+                        hi = mid;
+                }
+                if (lo < l1 && in_jump[lo] == j) {
+                    const int ep = m_short ? e : lo, eq = m_short ? lo : e;
+                    const double c = scale * in_coef[ep] * in_coef[eq];
+                    const double2 g = X[(int64_t)in_src[ep] * D + in_src[eq]];
+                    sx = fma(c, g.x, sx);
+                    sy = fma(c, g.y, sy);
+                }
             }
         }
         for (int off = 16; off > 0; off >>= 1) {

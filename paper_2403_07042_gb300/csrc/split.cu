@@ -397,26 +397,27 @@ __device__ __noinline__ bool long_merge_df(uint32_t *err, int64_t D, const int32
                 sr = __fmaf_rn(c.hi, ur, __fmaf_rn(c.lo, ur, sr));
                 si = __fmaf_rn(c.hi, ui, __fmaf_rn(c.lo, ui, si));
             }
-        } else
-        for (int e = s0 + lane; e < s1; e += 32) {
-            const int j = in_jump[e];
-            int lo = l0, hi = l1;  // first entry of the longer list with jump >= j
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (in_jump[mid] < j)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            const int ep = m_short ? e : lo, eq = m_short ? lo : e;  // row m's entry, row n's
-            if (lo < l1 && in_jump[lo] == j &&
-                qed_check(err, in_src[ep] >= 0 && in_src[ep] < D && in_src[eq] >= 0 && in_src[eq] < D)) {
-                const float2 cp = coef[ep], cq = coef[eq];
-                const df c = df_mul({cp.x, cp.y}, {cq.x, cq.y});
-                const float4 u = X[(int64_t)in_src[ep] * D + in_src[eq]];
-                const float ur = u.x + u.y, ui = u.z + u.w;
-                sr = __fmaf_rn(c.hi, ur, __fmaf_rn(c.lo, ur, sr));
-                si = __fmaf_rn(c.hi, ui, __fmaf_rn(c.lo, ui, si));
+        } else {
+            for (int e = s0 + lane; e < s1; e += 32) {
+                const int j = in_jump[e];
+                int lo = l0, hi = l1;  // first entry of the longer list with jump >= j
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (in_jump[mid] < j)
+                        lo = mid + 1;
+                    else
+                        hi = mid;
+                }
+                const int ep = m_short ? e : lo, eq = m_short ? lo : e;  // row m's entry, row n's
+                if (lo < l1 && in_jump[lo] == j &&
+                    qed_check(err, in_src[ep] >= 0 && in_src[ep] < D && in_src[eq] >= 0 && in_src[eq] < D)) {
+                    const float2 cp = coef[ep], cq = coef[eq];
+                    const df c = df_mul({cp.x, cp.y}, {cq.x, cq.y});
+                    const float4 u = X[(int64_t)in_src[ep] * D + in_src[eq]];
+                    const float ur = u.x + u.y, ui = u.z + u.w;
+                    sr = __fmaf_rn(c.hi, ur, __fmaf_rn(c.lo, ur, sr));
+                    si = __fmaf_rn(c.hi, ui, __fmaf_rn(c.lo, ui, si));
+                }
             }
         }
         for (int off = 16; off > 0; off >>= 1) {
@@ -484,57 +485,57 @@ __device__ __forceinline__ void lindblad_jt(const TileItem *__restrict__ tiles, 
     const float4 *X = X_only ? X_only : state_buf(a, xsel);
     const float4 *B = X_only ? nullptr : state_buf(a, bsel);
     float4 *O = X_only ? O_only : state_buf(a, osel);
-            // incoming entries by jump: element (m, n) gets c_j(m) c_j(n) X[src_j(m), src_j(n)] for
-            // every jump j with an entry in both rows (row entries warp-uniform, column entries
-            // read once for the thread's kRows rows)
-            const int nj = a.nj;
-            int4 tn[kInMax], tm[kRows][kInMax];
-            float2 dm[kRows];
-    #pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                const int64_t m = m0 + 8 * r, mc = m < D ? m : 0;
-                dm[r] = a.damp[mc];
-    #pragma unroll
-                for (int j = 0; j < kInMax; ++j)
-                    tm[r][j] = j < nj ? a.jtab[mc * kInMax + j] : make_int4(-1, 0, 0, 0);
-            }
-    #pragma unroll
-            for (int j = 0; j < kInMax; ++j) tn[j] = j < nj ? a.jtab[nc * kInMax + j] : make_int4(-1, 0, 0, 0);
-            pdl_wait();
-            pdl_trigger();
-            float4 v[kRows], u[kRows][kInMax], bv[kRows];
-    #pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                const int64_t m = m0 + 8 * r;
-                const bool inside = m < D && n_in;
-                v[r] = X[(inside ? m : 0) * D + nc];
-                // the base of a Strang stage comes with the gathers
-                bv[r] = B ? B[(inside ? m : 0) * D + nc] : make_float4(0.f, 0.f, 0.f, 0.f);
-    #pragma unroll
-                for (int j = 0; j < kInMax; ++j) {
-                    const bool hit = inside && tm[r][j].x >= 0 && tn[j].x >= 0 &&
-                                     qed_check(a.err, tm[r][j].x < D && tn[j].x < D);
-                    u[r][j] = hit ? X[(int64_t)tm[r][j].x * D + tn[j].x] : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-    #pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                const int64_t m = m0 + 8 * r;
-                if (!(m < D && n_in)) continue;
-                const cdf vv = load_cdf(v[r]);
-                float gr, gi;
-                damping_term(dm[r], dn, vv, gr, gi);
-    #pragma unroll
-                for (int j = 0; j < kInMax; ++j) {
-                    if (!(tm[r][j].x >= 0 && tn[j].x >= 0)) continue;
-                    const df c = df_mul({__int_as_float(tm[r][j].y), __int_as_float(tm[r][j].z)},
-                                        {__int_as_float(tn[j].y), __int_as_float(tn[j].z)});
-                    const float ur = u[r][j].x + u[r][j].y, ui = u[r][j].z + u[r][j].w;
-                    gr = __fmaf_rn(c.hi, ur, __fmaf_rn(c.lo, ur, gr));
-                    gi = __fmaf_rn(c.hi, ui, __fmaf_rn(c.lo, ui, gi));
-                }
-                                lindblad_store(a, O, m, n, load_cdf(bv[r]), f * gr, f * gi, planes);
-            }
+    // incoming entries by jump: element (m, n) gets c_j(m) c_j(n) X[src_j(m), src_j(n)] for
+    // every jump j with an entry in both rows (row entries warp-uniform, column entries
+    // read once for the thread's kRows rows)
+    const int nj = a.nj;
+    int4 tn[kInMax], tm[kRows][kInMax];
+    float2 dm[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int64_t m = m0 + 8 * r, mc = m < D ? m : 0;
+        dm[r] = a.damp[mc];
+#pragma unroll
+        for (int j = 0; j < kInMax; ++j)
+            tm[r][j] = j < nj ? a.jtab[mc * kInMax + j] : make_int4(-1, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < kInMax; ++j) tn[j] = j < nj ? a.jtab[nc * kInMax + j] : make_int4(-1, 0, 0, 0);
+    pdl_wait();
+    pdl_trigger();
+    float4 v[kRows], u[kRows][kInMax], bv[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int64_t m = m0 + 8 * r;
+        const bool inside = m < D && n_in;
+        v[r] = X[(inside ? m : 0) * D + nc];
+        // the base of a Strang stage comes with the gathers
+        bv[r] = B ? B[(inside ? m : 0) * D + nc] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < kInMax; ++j) {
+            const bool hit = inside && tm[r][j].x >= 0 && tn[j].x >= 0 &&
+                             qed_check(a.err, tm[r][j].x < D && tn[j].x < D);
+            u[r][j] = hit ? X[(int64_t)tm[r][j].x * D + tn[j].x] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int64_t m = m0 + 8 * r;
+        if (!(m < D && n_in)) continue;
+        const cdf vv = load_cdf(v[r]);
+        float gr, gi;
+        damping_term(dm[r], dn, vv, gr, gi);
+#pragma unroll
+        for (int j = 0; j < kInMax; ++j) {
+            if (!(tm[r][j].x >= 0 && tn[j].x >= 0)) continue;
+            const df c = df_mul({__int_as_float(tm[r][j].y), __int_as_float(tm[r][j].z)},
+                                {__int_as_float(tn[j].y), __int_as_float(tn[j].z)});
+            const float ur = u[r][j].x + u[r][j].y, ui = u[r][j].z + u[r][j].w;
+            gr = __fmaf_rn(c.hi, ur, __fmaf_rn(c.lo, ur, gr));
+            gi = __fmaf_rn(c.hi, ui, __fmaf_rn(c.lo, ui, gi));
+        }
+            lindblad_store(a, O, m, n, load_cdf(bv[r]), f * gr, f * gi, planes);
+    }
 }
 
 // The jump terms of element (m, n) from the incoming lists, added to (gr, gi): long pairs of lists by
