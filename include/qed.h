@@ -280,8 +280,8 @@ qed_status qed_evolve(qed_model *m, void *rho, int64_t n_steps, int64_t step_off
  * M = sum_n E(rho_n) U^+ kappa_n, and the rate gradients of both half steps (in split
  * precision the backward model runs the same stages; the forward pass keeps rho_n, E(rho_n)
  * and V_n of a segment).  QED_SCHEME_EFFECTIVE is not differentiated (EUNSUPPORTED).  In split precision rho0 must be Hermitian with unit trace (EINVAL otherwise, as
- * in qed_evolve).  The model keeps the work space for the next call while all models of the
- * process keep at most 2 GiB (qed_free returns it); synchronises `stream`.
+ * in qed_evolve).  The model keeps a work space of at most 2 GiB for the next call while all
+ * models of the process keep at most 8 GiB (qed_free returns it); synchronises `stream`.
  */
 qed_status qed_adjoint(qed_model *m, const void *rho0, int64_t n_steps, int32_t checkpoint_every,
                        const double *obs_diag, double *loss, double *grad_g, double *grad_zeta,
