@@ -119,8 +119,8 @@ struct SplitState {
     int4 *jtab = nullptr;                    // per-jump incoming table (at most kInMax jumps)
     int nj = 0;
     double scale_delta = 1.0, scale_rho = 1.0, scale_w = 1.0;
-    uint8_t *stats = nullptr;                // scratch of delta_stats_kernel
-    std::vector<uint8_t> nz;                 // [ceil(D / 64)]^2: blocks of Delta with a nonzero
+    uint8_t *stats = nullptr;                // scratch of delta_stats_kernel and delta_blocks_kernel
+    std::vector<uint8_t> nz;                 // [ceil(D / 64)]^2: blocks of Delta's planes with a nonzero
     int batch_bn1 = 0, batch_bn2 = 0;  // tile widths of the grouped launches (tuned or set), 0 by size
 };
 
@@ -153,14 +153,11 @@ __global__ void make_delta_kernel(int64_t D, const double2 *U, const double2 *P,
     Dl[idx] = d;
 }
 
-// What the planes' scales and the products' work lists need of Delta, one block per row:
-// stats = {max |Delta_kl|, max_k sum_l |Delta_kl|} (as bits: non-negative doubles order like
-// integers), nz[k / 64][l / 64] whether that block has a nonzero.
-__global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const double2 *Dl, unsigned long long *stats,
-                                                          uint8_t *nz) {
+// What the planes' scales need of Delta, one block per row: stats = {max |Delta_kl|,
+// max_k sum_l |Delta_kl|} (as bits: non-negative doubles order like integers).
+__global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const double2 *Dl, unsigned long long *stats) {
     __shared__ double part[2][8];
     const int64_t k = blockIdx.x;
-    const int64_t nb = (D + 63) / 64;
     double top = 0.0, sum = 0.0;
     for (int64_t l = threadIdx.x; l < D; l += blockDim.x) {
         const double2 d = Dl[k * D + l];
@@ -168,7 +165,6 @@ __global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const doubl
         if (!(x <= HUGE_VAL)) x = HUGE_VAL;  // NaN counts as infinity
         top = fmax(top, x);
         sum += x;
-        if (d.x != 0.0 || d.y != 0.0) nz[(k / 64) * nb + l / 64] = 1;
     }
     for (int off = 16; off > 0; off >>= 1) {
         top = fmax(top, __shfl_xor_sync(0xffffffffu, top, off));
@@ -186,6 +182,19 @@ __global__ void __launch_bounds__(256) delta_stats_kernel(int64_t D, const doubl
     }
     atomicMax(&stats[0], (unsigned long long)__double_as_longlong(top));
     atomicMax(&stats[1], (unsigned long long)__double_as_longlong(sum));
+}
+
+// nz[k / 64][l / 64]: whether the planes of that block of s Delta have a nonzero (one block per row).
+// An element whose leading FP16 piece is zero is zero in all three.  Delta reaches as far as the
+// couplings do in the series' terms, its planes only to 2^-39 of its largest element: with lists of
+// Delta's own nonzeros the 32 x 32 lattice's GEMM1 takes 100 us and GEMM2 88, with the planes' 75 and 76.
+__global__ void __launch_bounds__(256) delta_blocks_kernel(int64_t D, const double2 *Dl, double s, uint8_t *nz) {
+    const int64_t k = blockIdx.x, nb = (D + 63) / 64;
+    for (int64_t l = threadIdx.x; l < D; l += blockDim.x) {
+        const double2 d = Dl[k * D + l];
+        if (__half2float(__double2half(d.x * s)) != 0.f || __half2float(__double2half(d.y * s)) != 0.f)
+            nz[(k / 64) * nb + l / 64] = 1;
+    }
 }
 
 // a1 = [[Dre, Dim], [Dim, -Dre]] and b2 = [[Dre, Dim], [-Dim, Dre]] (2Dp x 2Dp) as three
@@ -931,11 +940,12 @@ bool plan_products(SplitState &S, TcGemm &g1, TcGemm &g2, int splits1, int bn1, 
            tc_gemm_plan(g2, S.w_pl, 2, S.b2, 3, Dp, 2 * Dp, 2 * Dp, 3, kSeg2Pairs, S.num_sms, splits2, bn2, true);
 }
 
-// The k-blocks of each tile of a product in which Delta's rows of that tile have a nonzero: Delta is
-// block diagonal over the components of H's graph (a chain's states are sorted by excitations), and
-// its padding is zero.  The blocks left out would add zeros, so nothing changes in the sums.  Tiles
-// hold `rows` rows of Delta each; K = [re | im], Dp columns each, in slices of g.kb_per_split
-// blocks, every one of which keeps at least one block.  Appends kb_ptr and kb_idx to `out`.
+// The k-blocks of each tile of a product in which the planes of Delta's rows of that tile have a
+// nonzero: Delta is block diagonal over the components of H's graph (a chain's states are sorted by
+// excitations), far elements round to zero, and its padding is zero.  The blocks left out would add
+// zeros, so nothing changes in the sums.  Tiles hold `rows` rows of Delta each; K = [re | im], Dp
+// columns each, in slices of g.kb_per_split blocks, every one of which keeps at least one block.
+// Appends kb_ptr and kb_idx to `out`.
 void k_block_lists(const std::vector<uint8_t> &nz, int64_t D, int64_t Dp, const TcGemm &g, int tiles, int rows,
                    std::vector<int> &out, size_t &ptr_at, size_t &idx_at) {
     const int nb = (int)((D + 63) / 64), half = (int)(Dp / 64), total = g.K / kTcBK;
@@ -1293,21 +1303,21 @@ qed_status split_prepare(qed_model *m, cudaStream_t s) {
     count_launches(1);
     const int64_t nb = (D + 63) / 64;
     QED_CUDA_TRY(cudaMemsetAsync(S.stats, 0, (size_t)(16 + nb * nb), s));
-    delta_stats_kernel<<<(unsigned)D, 256, 0, s>>>(D, m->work1, (unsigned long long *)S.stats, S.stats + 16);
-    count_launches(1);
-    std::vector<uint8_t> h((size_t)(16 + nb * nb));
-    QED_CUDA_TRY(cudaMemcpyAsync(h.data(), S.stats, h.size(), cudaMemcpyDeviceToHost, s));
+    delta_stats_kernel<<<(unsigned)D, 256, 0, s>>>(D, m->work1, (unsigned long long *)S.stats);
+    double top[2];  // largest element, largest row sum
+    QED_CUDA_TRY(cudaMemcpyAsync(top, S.stats, sizeof(top), cudaMemcpyDeviceToHost, s));
     QED_CUDA_TRY(cudaStreamSynchronize(s));
-    double maxabs = 0.0, maxrow = 0.0;
-    std::memcpy(&maxabs, h.data(), 8);
-    std::memcpy(&maxrow, h.data() + 8, 8);
     // largest scaled magnitude 2^14 (FP16 max 65504); |rho_kl| <= 1, |W_kl| <= max row sum of |Delta|
     const double scale_delta = S.scale_delta, scale_w = S.scale_w;
-    std::vector<uint8_t> nz(h.begin() + 16, h.end());
-    S.nz.swap(nz);
-    S.scale_delta = pow2_scale(maxabs, 14);
+    S.scale_delta = pow2_scale(top[0], 14);
     S.scale_rho = std::ldexp(1.0, 14);
-    S.scale_w = pow2_scale(maxrow, 14);
+    S.scale_w = pow2_scale(top[1], 14);
+    delta_blocks_kernel<<<(unsigned)D, 256, 0, s>>>(D, m->work1, S.scale_delta, S.stats + 16);
+    count_launches(2);
+    std::vector<uint8_t> nz((size_t)(nb * nb));
+    QED_CUDA_TRY(cudaMemcpyAsync(nz.data(), S.stats + 16, nz.size(), cudaMemcpyDeviceToHost, s));
+    QED_CUDA_TRY(cudaStreamSynchronize(s));
+    S.nz.swap(nz);
     // the last that may run out of memory; the tables are written once it has not
     qed_model *self[1] = {m};
     const qed_status st = build_batch(S.self, self, 1, true);
