@@ -418,7 +418,8 @@ __global__ void gather_kernel(int64_t D, const double2 *rho, int64_t n, const in
 
 // rho = V (1 - dt/2 (d_m + d_n)) + dt (jump terms).  Bound by FP64 issue: about 4 instructions an
 // element and 4 a jump term (11 us alone at dim 512).  The rows' tables are read before the wait on
-// the pass that writes V: 10 steps at dim 512 take 456 us, with plain launches and lists 482.
+// the pass that writes V, and jumps found by masks: 2.6 us a step less at dim 512 than with plain
+// launches and lists.
 __global__ void __launch_bounds__(256) dissipate_f64_kernel(int64_t D, const double2 *V, double2 *rho,
                                                             const double *__restrict__ anti, JumpLists l, double dt) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -4,7 +4,7 @@
 //
 // Every H of this library couples a basis state to a few others (one term per atom, bond and
 // tunnelling digit), so X t costs a few multiply-adds per element where the dense product
-// costs D: at dim 512 (at most five couplings a row, six terms) 1/40 of the multiply-adds.
+// costs D: at dim 512 (at most five couplings a row, seven terms) 1/25 of the multiply-adds.
 // The series starts from X' = X - Lambda, Lambda the middle of H's diagonal over each connected
 // component of H's graph: X is block diagonal over the components, so exp(X) =
 // exp(Lambda) exp(X') exactly, and what is left in X' (couplings and detunings) is small: a

@@ -584,10 +584,10 @@ __device__ __noinline__ void list_terms(const InstDesc &a, const float4 *X, int6
 // ranges of their jumps overlap: a lattice's only such element is the vacuum's population, which
 // the warp sums entry by entry.  The next row's elements are loaded before a row is worked on.
 // What bounds it: the 40 B an element streams (V 16, rho 16, planes 8) and the latency of the
-// gathers; large blocks (64 rows where that leaves eight blocks an SM) pay the staging once for
-// 4096 elements.  Measured alone from a cold L2: the 32 x 32 lattice 74 -> 45 us,
-// the 24 x 24 lattice's 34 -> 21 us, 64 chains of 32 to 1024 states 504 -> 300 us (the version that
-// merged its lists in registers, at 126 registers and two blocks an SM).
+// gathers (41 % issue, 2.6 TB/s on the 32 x 32 lattice); large blocks (64 rows where that leaves
+// eight blocks an SM) pay the staging once for 4096 elements.  Measured alone from a cold L2: the 32 x
+// 32 lattice 45 us (80 by the version that merged its lists in registers, two blocks an SM), 64 chains
+// of 32 to 1024 states 303 us.
 template <bool LIE>
 __device__ __forceinline__ void lindblad_update(const TileItem *__restrict__ tiles,
                                                 const InstDesc *__restrict__ descs, int rows, int xsel, int bsel,
