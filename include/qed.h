@@ -55,7 +55,11 @@ typedef enum {
 } qed_status;
 
 typedef enum {
-    QED_FP64 = 0,          /* U rho U^+ in FP64, through the sparse H or as two products   */
+    QED_FP64 = 0,          /* U rho U^+ in FP64, through the sparse H or as two products;
+                              a step through the sparse H ends its series where the tail is
+                              an FP64 rounding of what two couplings make, so that in one
+                              step elements four and more couplings away have the accuracy
+                              of the truncated series, not of their own size               */
     QED_SPLIT_FP16x2 = 1,  /* increment form on tcgen05: FP16 hi+lo operands, FP32 accumulate */
     QED_SPLIT_BF16x3 = 2,  /* reserved                                                    */
     QED_SPLIT_TF32x3 = 3   /* reserved                                                    */

@@ -24,8 +24,9 @@ namespace qed {
 struct SparseX {
     void *block = nullptr;       // the allocation of every table
     int D = 0;
-    int terms = 0;               // Taylor terms of exp(X' / substeps) in a pass, exact in small elements too
-    int frechet_terms = 0;       // of the Frechet derivative's series
+    int terms = 0;               // Taylor terms of exp(X' / substeps) in a step's pass
+    int all_terms = 0;           // in U's, at least 16
+    int frechet_terms = 0;       // of the Frechet derivative's series, at least 13
     int substeps = 0;
     double norm = 0.0;           // infinity norm of X'
     bool pays = false;           // a step is faster through it (passes_pay)
@@ -39,7 +40,7 @@ struct SparseX {
     int2 *order = nullptr;       // [D] {row, couplings}
     int *place = nullptr;        // [D] the sorted place of row k
     int4 *entry = nullptr;       // [longest row, at least 1][D] {column's place, 0, dt H_kl}
-    double *inv = nullptr;       // [terms + 1] 1 / (substeps n)
+    double *inv = nullptr;       // [all_terms + 1] 1 / (substeps n)
     double2 *diag_sorted = nullptr;  // [D] diag in sorted order, or null
     // Lambda's distinct values: class of each row, and phi of class a times conj(phi) of b
     int *cls = nullptr;          // [D]

@@ -468,3 +468,32 @@ def test_fp64_passes_of_the_largest_dimensions(shape):
     gm.sync()
     assert (rho - torch.outer(psi, psi.conj())).abs().max().item() <= 96 * U
     assert "strip_f64_1" in gm.profile(rho, 1)
+
+
+@pytest.mark.parametrize("D,precision", [(64, "fp64"), (129, "fp64"), (129, "split_fp16x2")])
+@pytest.mark.parametrize("detuned", [False, True])
+@pytest.mark.parametrize("dt", [0.1, 1e-3])
+def test_propagator_is_exact_many_couplings_away(D, precision, detuned, dt):
+    """Elements up to eight couplings away, as the Pade approximant has them: 11 u a level and the
+    phases' 7 u (as for second neighbours above), the series' tail far below: 11 h + 16 u."""
+    m = chain(D, detuned, dt)
+    H = np.asarray(qed.spec_hamiltonian(m)).real
+    X = H.astype(np.longdouble) * np.longdouble(dt)
+    re, im, term = np.eye(D, dtype=np.longdouble), np.zeros((D, D), np.longdouble), np.eye(D, dtype=np.longdouble)
+    for n in range(1, 40):
+        term = X @ term / n
+        if n % 2:
+            im += (-1) ** ((n + 1) // 2) * term
+        else:
+            re += (-1) ** (n // 2) * term
+    near = ((H != 0) | (np.eye(D) > 0)).astype(int)
+    got = qed.Model(m, precision=precision).get_U().cpu().numpy()
+    err = np.hypot((got.real - re).astype(float), (got.imag - im).astype(float))
+    size = np.hypot(re.astype(float), im.astype(float))
+    reach, before = near > 0, np.eye(D) > 0
+    for h in range(1, 9):
+        at = reach & ~before
+        if at.any():
+            assert (err[at] / size[at]).max() <= (11 * h + 16) * U, (h, (err[at] / size[at]).max() / U)
+        before, reach = reach, reach.astype(int) @ near > 0
+    assert at.any()
